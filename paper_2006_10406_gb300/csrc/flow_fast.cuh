@@ -69,12 +69,11 @@ __global__ void __launch_bounds__(256, 4) fsi_flow_fast(const __grid_constant__ 
     __shared__ double red[64];
     __shared__ int s_pair[5];  // cycle of this launch (negative: none left), step, tile column and row; ready
     const StepArgs<float> &p = a.s;
-    if (p.ctl->done) return;
     float *su = sm, *sx = su + G::SU_W * G::SU_H, *ss = sx + G::SXT;
     const int tid = threadIdx.x, w = p.w, h = p.h;
     const long pitch = p.pitch;
     const int ntx = (w + 63) / 64, nty = (h + TH - 1) / TH, ntiles = ntx * nty;
-    const int cycle0 = p.ctl->cycles;
+    const int cycle0 = a.cycle0;
     auto decode = [&](const unsigned int t) {
         const int step = (int)(t / (unsigned)ntiles), tile = (int)(t - (unsigned)step * ntiles);
         const int c = step / a.n;
@@ -83,8 +82,15 @@ __global__ void __launch_bounds__(256, 4) fsi_flow_fast(const __grid_constant__ 
         s_pair[3] = tile / ntx;
         s_pair[2] = tile - s_pair[3] * ntx;
     };
-    // warp 0 hands out pairs, warp 1 stores the flags
-    if (tid == 0) decode(atomicAdd(a.ticket, 1u));
+    // warp 0 hands out pairs, warp 1 stores the flags. A CTA may start after others have ended
+    // cycles, so what they store in the control block is looked at by one thread only, and the
+    // launch's first cycle is an argument.
+    if (tid == 0) {
+        if (*(volatile const int *)&p.ctl->done || *(volatile const int *)&p.ctl->timeout)
+            s_pair[0] = -1;
+        else
+            decode(atomicAdd(a.ticket, 1u));
+    }
     __syncthreads();
     for (;;) {
         const int c = s_pair[0], k = s_pair[1], tx = s_pair[2], ty = s_pair[3];

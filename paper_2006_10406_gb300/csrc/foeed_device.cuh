@@ -104,6 +104,7 @@ struct FlowArgs {
     unsigned int *ticket;  // next (step, tile) of this launch
     int *done;             // per tile: steps of the solve completed
     int n, cycles;         // steps per cycle, cycles of this launch
+    int cycle0;            // cycles of the solve before this launch
     float alpha[kCycleMax], alpha_lo[kCycleMax];
 };
 

@@ -4,6 +4,7 @@ at the edges of its tiles and of its dispatch rule.
 Tolerances: one FP64 step 1e-12, one FP32 step 2e-5 (float rounding of |tau P u| <=
 tau * 32 * max|u|), as in test_gpu_parity.py."""
 import ctypes as C
+import threading
 
 import numpy as np
 import pytest
@@ -344,6 +345,49 @@ def test_flow_solve_stops_where_it_diverges():
     a, b = _both(0, f, m, 0.05, 1.0, 20, 50, tau=0.4)
     assert a[1].status == 4 and a[1].cycles_run == b[1].cycles_run
     np.testing.assert_array_equal(a[0].cpu().numpy(), b[0].cpu().numpy())
+
+
+def test_flow_solves_beside_other_streams_match_sequential_solves():
+    """Two threads with a stream each while a third stream's kernels come and go: CTAs of a cooperative launch may
+    start after others have ended cycles."""
+    cases = [(0, 2, 150, {}), (1, 3, 100, dict(tol=1e-4)), (0, 2, 120, dict(dtype="f32_f64u"))]
+    images = [_image(1000, 1300, seed=5), _image(840, 1100, seed=6)]
+
+    def solve(f, m, case, **kw):
+        method, n, cycles, opt = case
+        fn = fg.foeed_inpaint if method == 0 else fg.eed_inpaint
+        return fn(f, m, 0.05, 1.0, n, cycles, raise_on_status=False, **opt, **kw)
+
+    ref = [[solve(f, m, c) for c in cases] for f, m in images]
+    torch.cuda.synchronize(DEV)
+    got, errors = {}, []
+
+    def worker(i):
+        try:
+            s = torch.cuda.Stream(device=DEV)
+            for rep in range(3):
+                for j, c in enumerate(cases):
+                    got[i, rep, j] = solve(*images[i], c, stream=s)
+            s.synchronize()
+        except Exception as e:  # reported below
+            errors.append(e)
+
+    other = torch.cuda.Stream(device=DEV)
+    buf = torch.ones(1 << 26, device=DEV)
+    other.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(other):
+        for _ in range(400):  # some 40 ms of kernels that fill the GPU
+            buf.mul_(1.0)
+    ts = [threading.Thread(target=worker, args=(i,)) for i in range(2)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize(DEV)
+    assert not errors, errors
+    assert len(got) == 2 * 3 * len(cases)
+    for (i, rep, j), a in got.items():
+        _same(a, ref[i][j])
 
 
 # --------------------------------------------------------------------------
