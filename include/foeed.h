@@ -332,7 +332,7 @@ foeed_status foeed_set_tile_policy(int policy);
  * calling thread. Times are microseconds per FSI step measured by the autotuner
  * (0 when it did not run for that solve, e.g. a cached or fixed choice). */
 typedef struct {
-    int tile_h;      /* single image: 64, 32, 16 or 8 (0: the generic kernel ran); batch: 0 */
+    int tile_h;      /* single image: 64, 32, 16 or 8 (24: reported as 32; 0: FP64 or the generic kernel); batch: 0 */
     int images;      /* images in the solve */
     int images_h16;  /* images solved on 64 x 16 tiles */
     int tuned;       /* 1 if the autotuner timed the candidates for this solve */
@@ -343,6 +343,24 @@ typedef struct {
     float us_h8;     /* single FOEED image: time with 64 x 8 tiles (0 otherwise) */
 } foeed_tile_plan;
 foeed_status foeed_last_tile_plan(foeed_tile_plan *out);
+
+/* How the last foeed_inpaint / eed_inpaint / foeed_inpaint_states on the calling thread ran. */
+typedef enum {
+    FOEED_ROUTE_STEPS = 0,    /* a captured graph per cycle, one launch per step */
+    FOEED_ROUTE_RESIDENT = 1, /* cooperative launches of many cycles, every tile resident */
+    FOEED_ROUTE_ORDERED = 2   /* cooperative launches of many cycles, tiles taken in order */
+} foeed_route_kind;
+typedef struct {
+    int kind;           /* foeed_route_kind of the launches that made the result */
+    int tile_w, tile_h; /* their tiles (0: steps in FP64 or on the generic kernel) */
+    int gave_up;        /* 1: a cooperative launch's wait ran out and the solve was repeated step by step */
+} foeed_route;
+foeed_status foeed_last_route(foeed_route *out);
+
+/* Polls after which a wait inside a cooperative launch gives up (0: the default, some half a
+ * second), for later solves of the calling thread. A solve that gives up leaves u_inout as it
+ * was and is repeated step by step, with the same result. FOEED_ERR_ARG for a negative number. */
+foeed_status foeed_set_wait_limit(int polls);
 
 /* Message describing the last failure on the calling thread ("" if none). */
 const char *foeed_last_error(void);

@@ -26,7 +26,7 @@ from . import build as _build
 __all__ = ["foeed_inpaint", "eed_inpaint", "foeed_inpaint_batch", "eed_inpaint_batch", "inpaint_channels",
            "foeed_inpaint_vjp", "foeed_inpaint_diff",
            "foeed_step", "eed_step", "foeed_errors", "foeed_apply_tensor_field", "workspace_bytes",
-           "set_tile_policy", "last_tile_plan",
+           "set_tile_policy", "last_tile_plan", "last_route", "set_wait_limit",
            "Report", "FoeedError", "lib", "F32", "F64", "F32_F64U", "STATUS"]
 
 F32, F64, F32_F64U = 0, 1, 2
@@ -64,6 +64,11 @@ class _TilePlan(C.Structure):
                 ("us_h8", C.c_float)]
 
 
+class _Route(C.Structure):
+    _fields_ = [("kind", C.c_int), ("tile_w", C.c_int), ("tile_h", C.c_int), ("gave_up", C.c_int)]
+
+
+ROUTE = {0: "steps", 1: "resident", 2: "ordered"}
 TILE_POLICY = {"auto": 0, "h8": 8, "h16": 16, "h32": 32, "h64": 64, 0: 0, 8: 8, 16: 16, 32: 32, 64: 64}
 
 
@@ -127,6 +132,10 @@ def lib():
         L.foeed_set_tile_policy.restype = i
         L.foeed_last_tile_plan.argtypes = [C.POINTER(_TilePlan)]
         L.foeed_last_tile_plan.restype = i
+        L.foeed_last_route.argtypes = [C.POINTER(_Route)]
+        L.foeed_last_route.restype = i
+        L.foeed_set_wait_limit.argtypes = [i]
+        L.foeed_set_wait_limit.restype = i
         L.foeed_last_error.restype = C.c_char_p
         L.foeed_version.restype = C.c_char_p
         _lib = L
@@ -209,6 +218,20 @@ def last_tile_plan():
     t = _TilePlan()
     _check(lib().foeed_last_tile_plan(C.byref(t)))
     return {k: getattr(t, k) for k, _ in _TilePlan._fields_}
+
+
+def last_route():
+    """How the last solve on this thread ran: kind ("steps", "resident" or "ordered"), tile_w, tile_h and
+    gave_up (a cooperative launch's wait ran out and the solve was repeated step by step)."""
+    r = _Route()
+    _check(lib().foeed_last_route(C.byref(r)))
+    return {"kind": ROUTE[r.kind], "tile_w": r.tile_w, "tile_h": r.tile_h, "gave_up": bool(r.gave_up)}
+
+
+def set_wait_limit(polls=0):
+    """Polls after which a wait inside a cooperative launch gives up, for later solves on this host
+    thread (0: the default, some half a second)."""
+    _check(lib().foeed_set_wait_limit(int(polls)))
 
 
 def workspace_bytes(w, h, dtype=F32):

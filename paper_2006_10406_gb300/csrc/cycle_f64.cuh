@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kThreads) fsi_cycle_f64(const __grid_constant_
             }
         }
         if (last) {
-            if (m > 0 && !cycle_goes_on(p.ctl, cycle0 + m, &s_dead)) break;
+            if (m > 0 && !cycle_goes_on(p.ctl, cycle0 + m, &s_dead, a.poll0)) break;
             cycle_change(rnum, rden, p.ctl, p.partials, ntiles, bid, cycle0 + m + 1, red);
             ++m;
         }
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kThreads) fsi_cycle_f64(const __grid_constant_
         uint32_t pend = 0;
 #pragma unroll
         for (int j = 0; j < K; ++j) pend |= from[j] >= 0 ? 1u << j : 0u;
-        for (int it = 0; pend; ++it) {
+        for (int it = a.poll0; pend; ++it) {
             unsigned long long hi[K], lo[K];
 #pragma unroll
             for (int j = 0; j < K; ++j)

@@ -24,16 +24,13 @@
 // one (2.9 us a step with one launch per cycle of 25).
 //
 // It fits when all tiles are resident at once, which the cooperative launch guarantees.
-// Waits are bounded: a tile that does not see a tag within kPollLimit polls (about half a
-// second) raises ctl->timeout and leaves, and so do the others; the caller then runs the
-// step kernels.
+// Waits are bounded (kPollLimit): a tile that does not see a tag in time raises ctl->timeout
+// and leaves, and so do the others; the caller then runs the step kernels.
 #pragma once
 
 #include "step_fast.cuh"
 
 namespace foeed {
-
-constexpr int kPollLimit = 1 << 19;
 
 __device__ __forceinline__ void halo_store(unsigned long long *d, const float v, const uint32_t tag)
 {
@@ -113,10 +110,10 @@ __device__ __forceinline__ void halo_items(HaloItems<H::K> &q, const int w, cons
 // Gathers them from the words of step `tag` into su; false if a wait ran out.
 template <int K>
 __device__ __forceinline__ bool gather_halo(const HaloItems<K> &q, const unsigned long long *halo, const uint32_t tag,
-                                            float *su, const Ctl *ctl)
+                                            float *su, const Ctl *ctl, const int poll0)
 {
     uint32_t pend = q.used;
-    for (int it = 0; pend; ++it) {
+    for (int it = poll0; pend; ++it) {
         unsigned long long a[K], b[K];
 #pragma unroll
         for (int j = 0; j < K; ++j)
@@ -162,13 +159,13 @@ __device__ __forceinline__ void cycle_change(double rnum, double rden, Ctl *ctl,
 
 // Whether the solve goes on after cycle number `cycle`; waits for that verdict. A wait that
 // runs out raises *dead and stops.
-__device__ __forceinline__ bool cycle_goes_on(Ctl *ctl, const int cycle, int *dead)
+__device__ __forceinline__ bool cycle_goes_on(Ctl *ctl, const int cycle, int *dead, const int poll0)
 {
     __shared__ int s_on;
     __syncthreads();
     if (threadIdx.x == 0) {
         int v = 0;
-        for (int it = 0;; ++it) {
+        for (int it = poll0;; ++it) {
             v = *(volatile const int *)&ctl->verdict[cycle & 1];
             if (v == cycle || v == -cycle) break;
             if (it >= kPollLimit || ((it & 1023) == 1023 && *(volatile const int *)&ctl->timeout)) {
@@ -279,7 +276,7 @@ __global__ void __launch_bounds__(FastTile<R, EED, TH, LAT>::NTHR, FastTile<R, E
             }
         });
         if (last) {
-            if (m > 0 && !cycle_goes_on(p.ctl, cycle0 + m, &s_dead)) break;  // cycle m - 1 was the last one
+            if (m > 0 && !cycle_goes_on(p.ctl, cycle0 + m, &s_dead, a.poll0)) break;  // cycle m - 1 was the last one
             cycle_change(rnum, rden, p.ctl, p.partials, ntiles, bid, cycle0 + m + 1, red);
             ++m;
         }
@@ -293,7 +290,7 @@ __global__ void __launch_bounds__(FastTile<R, EED, TH, LAT>::NTHR, FastTile<R, E
                     for (int j = 0; j < 4; ++j)
                         if (x0 + 4 * qe + j < w) su[(re + e + G::HL) * G::SU_W + 4 * qe + 8 + j] = nu[e][j];
         }
-        if (!gather_halo(items, halo, tag, su, p.ctl)) {
+        if (!gather_halo(items, halo, tag, su, p.ctl, a.poll0)) {
             s_dead = 1;
             *(volatile int *)&p.ctl->timeout = 1;
         }

@@ -46,7 +46,7 @@ __device__ __forceinline__ bool flow_ready(const FlowArgs &a, const int ntx, con
     const bool flag = lane < 9 && nx >= 0 && nx < ntx && ny >= 0 && ny < nty;
     const int *src = flag ? a.done + ny * ntx + nx : &ctl->verdict[cycle & 1];
     bool ok = true, wait = flag || (lane == 9 && cycle > 0);
-    for (int it = 0; wait; ++it) {
+    for (int it = a.poll0; wait; ++it) {
         int v;
         asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(src) : "memory");
         wait = flag ? v < need : v != cycle && v != -cycle;

@@ -80,11 +80,15 @@ struct StepArgs {
 // FSI cycles of a small image in one cooperative launch (cycle_fast.cuh): step arguments
 // plus what the cycles add.
 constexpr int kCycleMax = 128;  // longest cycle (kernel parameter space)
+// A device wait gives up when its counter of polls passes kPollLimit at a multiple of 1024
+// (about half a second from 0); a host limit on the polls is a later start of the counter.
+constexpr int kPollLimit = 1 << 19;
 struct CycleArgs {
     StepArgs<float> s;         // mask, sizes, model, control block, partials (two sets)
     float *u[2];               // u[0]: u^{m,0} in, the last iterate out; u[1]: scratch
     unsigned long long *halo;  // two images of (value, tag) words, row pitch s.pitch
     int n, cycles;             // steps per cycle, cycles of this launch
+    int poll0;                 // start of the counters of polls
     float alpha[kCycleMax], alpha_lo[kCycleMax];
 };
 
@@ -93,7 +97,7 @@ struct CycleArgs64 {
     StepArgs<double> s;
     double *u[2];
     unsigned long long *halo;  // two words per pixel
-    int n, cycles;
+    int n, cycles, poll0;
     double alpha[kCycleMax];
 };
 
@@ -105,6 +109,7 @@ struct FlowArgs {
     int *done;             // per tile: steps of the solve completed
     int n, cycles;         // steps per cycle, cycles of this launch
     int cycle0;            // cycles of the solve before this launch
+    int poll0;             // start of the counters of polls
     float alpha[kCycleMax], alpha_lo[kCycleMax];
 };
 

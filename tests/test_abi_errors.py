@@ -175,3 +175,17 @@ def test_tile_policy_arguments_are_checked_on_the_host():
             fg.set_tile_policy("h128")
     finally:
         L.foeed_set_tile_policy(0)
+
+
+def test_route_query_and_wait_limit_arguments_are_checked_on_the_host():
+    import ctypes as C
+
+    import paper_2006_10406_gb300 as fg
+    L = fg.lib()
+    try:
+        assert L.foeed_last_route(None) == 1
+        assert L.foeed_last_route(C.byref(fg._Route())) == 0
+        assert L.foeed_set_wait_limit(-1) == 1 and b"wait limit" in L.foeed_last_error()
+        assert L.foeed_set_wait_limit(1) == 0
+    finally:
+        assert L.foeed_set_wait_limit(0) == 0

@@ -360,7 +360,7 @@ def test_flow_solves_beside_other_streams_match_sequential_solves():
 
     ref = [[solve(f, m, c) for c in cases] for f, m in images]
     torch.cuda.synchronize(DEV)
-    got, errors = {}, []
+    got, routes, errors = {}, [], []
 
     def worker(i):
         try:
@@ -368,6 +368,7 @@ def test_flow_solves_beside_other_streams_match_sequential_solves():
             for rep in range(3):
                 for j, c in enumerate(cases):
                     got[i, rep, j] = solve(*images[i], c, stream=s)
+                    routes.append(fg.last_route())
             s.synchronize()
         except Exception as e:  # reported below
             errors.append(e)
@@ -386,8 +387,60 @@ def test_flow_solves_beside_other_streams_match_sequential_solves():
     torch.cuda.synchronize(DEV)
     assert not errors, errors
     assert len(got) == 2 * 3 * len(cases)
+    assert all(r["kind"] == "ordered" and not r["gave_up"] for r in routes), routes
     for (i, rep, j), a in got.items():
         _same(a, ref[i][j])
+
+
+# --------------------------------------------------------------------------
+# the route of a solve, and a cooperative launch that gives up
+
+# method, keywords, shape, kind and tile
+ROUTES = [(0, {}, (250, 511), "resident", (64, 8)), (1, {}, (512, 515), "resident", (64, 16)),
+          (0, dict(dtype="f32_f64u"), (700, 701), "resident", (64, 16)), (0, {}, (720, 1280), "resident", (64, 24)),
+          (0, dict(diffusivity=1, mu3_mode=1), (300, 400), "resident", (64, 8)),
+          (0, dict(dtype="f64"), (64, 64), "resident", (8, 4)), (1, dict(dtype="f64"), (200, 200), "resident", (16, 16)),
+          (0, {}, (1000, 1300), "ordered", (64, 16)), (1, {}, (1080, 1920), "ordered", (64, 32)),
+          (0, dict(diffusivity=1), (1000, 1300), "steps", None), (0, dict(dtype="f64"), (512, 512), "steps", None),
+          (0, {}, (3000, 2900), "steps", None)]
+
+
+@pytest.mark.parametrize("method,kw,shape,kind,tile", ROUTES)
+def test_route_of_a_solve_and_of_one_that_gives_up(method, kw, shape, kind, tile):
+    """A wait limit of one poll: the kernel leaves with its status, and the solve is repeated step by step from its
+    inputs, u0 among them, with the same bits. Without cooperative launches the limit changes nothing."""
+    f, m = _image(*shape, seed=8)
+    kw = dict(kw, u0=torch.flip(f, (0,)))
+    a, b = _both(method, f, m, 0.05, 1.0, 12, 5, **kw)
+    solve = fg.foeed_inpaint if method == 0 else fg.eed_inpaint
+    again = solve(f, m, 0.05, 1.0, 12, 5, **kw)
+    route = fg.last_route()
+    assert (route["kind"], route["gave_up"]) == (kind, False)
+    assert tile is None or (route["tile_w"], route["tile_h"]) == tile
+    fg.set_wait_limit(1)
+    try:
+        c = solve(f, m, 0.05, 1.0, 12, 5, **kw)
+        route = fg.last_route()
+    finally:
+        fg.set_wait_limit(0)
+    assert (route["kind"], route["gave_up"]) == ("steps", kind != "steps")
+    for x in (a, again, c):
+        _same(x, b)
+
+
+def test_differentiable_solve_that_gives_up():
+    f, m = _image(300, 400, seed=9)
+    grads = []
+    for polls in (0, 1):
+        x = f.clone().requires_grad_(True)
+        fg.set_wait_limit(polls)
+        try:
+            u = fg.foeed_inpaint_diff(x, m, 0.05, 1.0, 10, 4)
+            assert fg.last_route()["gave_up"] == (polls == 1)
+        finally:
+            fg.set_wait_limit(0)
+        grads.append((u.detach(), torch.autograd.grad(u, x, torch.cos(7.0 * u.detach()))[0]))
+    assert torch.equal(grads[0][0], grads[1][0]) and torch.equal(grads[0][1], grads[1][1])
 
 
 # --------------------------------------------------------------------------
