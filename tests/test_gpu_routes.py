@@ -428,6 +428,20 @@ def test_route_of_a_solve_and_of_one_that_gives_up(method, kw, shape, kind, tile
         _same(x, b)
 
 
+def _kind(method, shape, sigma, n, cycles, **kw):
+    f, m = _image(*shape, seed=1)
+    (fg.foeed_inpaint if method == 0 else fg.eed_inpaint)(f, m, 0.05, sigma, n, cycles, raise_on_status=False, **kw)
+    return fg.last_route()["kind"]
+
+
+@pytest.mark.parametrize("method", [0, 1])
+@pytest.mark.parametrize("dtype,more", [("f32", "steps"), ("f32_f64u", "ordered")])
+def test_wide_gaussian_on_24_high_tiles_to_three_per_sm(method, dtype, more):
+    """456 tiles of 64 x 24 and 460, the same for both methods."""
+    assert _kind(method, (576, 1216), 2.0, 12, 2, dtype=dtype) == "resident"
+    assert _kind(method, (552, 1280), 2.0, 12, 2, dtype=dtype) == more
+
+
 def test_differentiable_solve_that_gives_up():
     f, m = _image(300, 400, seed=9)
     grads = []
