@@ -309,9 +309,13 @@ foeed_status foeed_inpaint_static(const void *f, const uint8_t *mask, void *u_in
  *     solved step by step). FP64 likewise (any diffusivity and mu3; up to three
  *     16 x 16 tiles per SM; tiles of 8 x 4, 8 x 8 or 16 x 16; 32 bytes per pixel).
  *     Larger FP32 images, to 4000 tiles of 64 x 32, mostly time nothing either (but for some
- *     of 609 to 836 tiles of 64 x 16 and a wide Gaussian): the steps of many cycles run in
- *     one cooperative launch of 64 x 16 (to 1400 of them) or 64 x 32 tiles taken in order (36
- *     bytes of workspace per 64 x 16 tile, included and optional in the same way).
+ *     of 609 to 836 tiles of 64 x 16 and a wide Gaussian, and plain FOEED with sigma under 2
+ *     beyond 3400): the steps of many cycles run in one cooperative launch of 64 x 16 (to 1400
+ *     of them) or 64 x 32 tiles taken in order (36 bytes of workspace per 64 x 16 tile, included
+ *     and optional in the same way), in cycles of at least six steps, ten a launch (from 912
+ *     tiles of 64 x 32: four, eight), and of at most 128. Shorter ones run step by step, as do
+ *     launches of under four steps on images of 305 to 608 tiles of 64 x 16. foeed_last_route
+ *     tells which.
  * The policy applies to the calling host thread's later calls: foeed_inpaint,
  * eed_inpaint and the batched solvers tune as above; foeed_step, eed_step,
  * foeed_inpaint_static and the forward steps of foeed_inpaint_vjp, which do

@@ -350,7 +350,7 @@ def test_flow_solve_stops_where_it_diverges():
 def test_flow_solves_beside_other_streams_match_sequential_solves():
     """Two threads with a stream each while a third stream's kernels come and go: CTAs of a cooperative launch may
     start after others have ended cycles."""
-    cases = [(0, 2, 150, {}), (1, 3, 100, dict(tol=1e-4)), (0, 2, 120, dict(dtype="f32_f64u"))]
+    cases = [(0, 6, 50, {}), (1, 7, 50, dict(tol=1e-4)), (0, 6, 40, dict(dtype="f32_f64u"))]
     images = [_image(1000, 1300, seed=5), _image(840, 1100, seed=6)]
 
     def solve(f, m, case, **kw):
@@ -440,6 +440,50 @@ def test_wide_gaussian_on_24_high_tiles_to_three_per_sm(method, dtype, more):
     """456 tiles of 64 x 24 and 460, the same for both methods."""
     assert _kind(method, (576, 1216), 2.0, 12, 2, dtype=dtype) == "resident"
     assert _kind(method, (552, 1280), 2.0, 12, 2, dtype=dtype) == more
+
+
+# n, cycles, route: few steps in a launch and short cycles are left to the step kernels
+@pytest.mark.parametrize("shape,n,cycles,kind", [
+    ((700, 701), 3, 1, "steps"), ((700, 701), 2, 2, "resident"), ((300, 400), 2, 1, "resident"),
+    ((1000, 1300), 5, 20, "steps"), ((1000, 1300), 9, 1, "steps"), ((1000, 1300), 6, 2, "ordered"),
+    ((1080, 1920), 3, 20, "steps"), ((1080, 1920), 4, 1, "steps"), ((1080, 1920), 4, 2, "ordered")])
+def test_route_by_the_number_of_steps(shape, n, cycles, kind):
+    f, m = _image(*shape, seed=n)
+    a, b = _both(0, f, m, 0.05, 1.0, n, cycles)
+    _same(a, b)
+    assert _kind(0, shape, 1.0, n, cycles) == kind
+
+
+@pytest.mark.parametrize("shape,n,kind", [((700, 701), 3, "steps"), ((700, 701), 4, "resident"), ((1000, 1300), 9, "steps"),
+                                          ((1000, 1300), 10, "ordered"), ((1080, 1920), 7, "steps"), ((1080, 1920), 8, "ordered")])
+def test_route_of_kept_states_by_the_cycle_length(shape, n, kind):
+    f, m = _image(*shape, seed=n)
+    x = f.clone().requires_grad_(True)
+    u = fg.foeed_inpaint_diff(x, m, 0.05, 1.0, n, 4)
+    assert fg.last_route()["kind"] == kind
+    (g,) = torch.autograd.grad(u, x, torch.ones_like(u))
+    ref, uref = fg.foeed_inpaint_vjp(f, m, torch.ones_like(f), 0.05, 1.0, n, 4)
+    assert torch.equal(u.detach(), uref) and torch.equal(g, ref)
+
+
+@pytest.mark.parametrize("method,kw,sigma,shape,kind", [
+    (0, {}, 1.5, (2176, 3200), "ordered"), (0, {}, 1.5, (2177, 3200), "steps"), (0, {}, 2.0, (2177, 3200), "ordered"),
+    (1, {}, 1.5, (2177, 3200), "ordered"), (0, dict(dtype="f32_f64u"), 1.0, (2177, 3200), "ordered")])
+def test_largest_ordered_solves(method, kw, sigma, shape, kind):
+    """3400 tiles of 64 x 32 and one row of tiles more."""
+    f, m = _image(*shape, seed=3)
+    _same(*_both(method, f, m, 0.05, sigma, 4, 2, **kw))
+    assert _kind(method, shape, sigma, 4, 2, **kw) == kind
+
+
+@pytest.mark.parametrize("method", [0, 1])
+# the edges of the ordered kernel's tiles (64 x 16, then 64 x 32) in cycles that it takes
+@pytest.mark.parametrize("shape", [(801, 1217), (33, 26801), (1008, 1400), (1009, 1400), (959, 1345), (33, 39050)])
+@pytest.mark.parametrize("sigma", [0.5, 2.0])
+def test_ordered_solve_at_tile_edges(method, shape, sigma):
+    f, m = _image(*shape, seed=shape[0])
+    _same(*_both(method, f, m, 0.05, sigma, 6, 3))
+    assert _kind(method, shape, sigma, 6, 3) == "ordered"
 
 
 def test_differentiable_solve_that_gives_up():
