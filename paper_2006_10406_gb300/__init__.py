@@ -451,9 +451,9 @@ def _autograd_function():
         the iterates at the start of every cycle where the forward kept them."""
 
         @staticmethod
-        def forward(ctx, f, mask, lam, sigma, cycle_len, max_cycles, tau, checkpoint_every):
+        def forward(ctx, f, mask, lam, sigma, cycle_len, max_cycles, tau, checkpoint_every, grad):
             ctx.cfg = (lam, sigma, cycle_len, max_cycles, tau, checkpoint_every)
-            if not (ctx.needs_input_grad[0] and _keeps_states(f, mask, cycle_len, max_cycles, checkpoint_every)):
+            if not (grad and ctx.needs_input_grad[0] and _keeps_states(f, mask, cycle_len, max_cycles, checkpoint_every)):
                 u, _ = foeed_inpaint(f.detach(), mask, lam, sigma, cycle_len, max_cycles, tau=tau)
                 ctx.save_for_backward(f.detach(), mask)
                 return u
@@ -484,7 +484,7 @@ def _autograd_function():
                     grad_u = _pitched_like(grad_u.to(f.dtype), pitch)
                 gf = torch.empty_strided(f.shape, (pitch, 1), dtype=f.dtype, device=f.device)
                 _states_call("grad", f, mask, lam, sigma, n, cycles, tau, states, grad_u, gf)
-            return gf, None, None, None, None, None, None, None
+            return gf, None, None, None, None, None, None, None, None
 
     return FoeedInpaint
 
@@ -498,7 +498,9 @@ def foeed_inpaint_diff(f, mask, lam, sigma, cycle_len, max_cycles, tau=0.0, chec
     global _FoeedInpaint
     if _FoeedInpaint is None:
         _FoeedInpaint = _autograd_function()
-    return _FoeedInpaint.apply(f, mask, lam, sigma, cycle_len, max_cycles, tau, checkpoint_every)
+    import torch
+    # needs_input_grad is true under torch.no_grad too, where no backward will follow
+    return _FoeedInpaint.apply(f, mask, lam, sigma, cycle_len, max_cycles, tau, checkpoint_every, torch.is_grad_enabled())
 
 
 def _step(method, u_prev, u_cur, u_next, mask, alpha, lam, sigma, tau=0.0, diffusivity=0, mu3_mode=0,

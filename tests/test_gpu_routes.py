@@ -525,6 +525,18 @@ def test_gradient_from_kept_states_is_the_vjp(shape, n, cycles, keep, dtype):
     assert torch.equal(u.detach(), uref) and torch.equal(g1, ref) and torch.equal(g2, ref)
 
 
+@pytest.mark.parametrize("mode", [torch.no_grad, torch.inference_mode, torch.enable_grad])
+def test_iterates_are_kept_only_where_a_gradient_is_recorded(mode, monkeypatch):
+    calls, states_call = [], fg._states_call
+    monkeypatch.setattr(fg, "_states_call", lambda *a: (calls.append(a[0]), states_call(*a)))
+    f, m = _image(70, 131, seed=2)
+    ref, _ = fg.foeed_inpaint(f, m, 0.05, 1.0, 10, 4)
+    x = f.clone().requires_grad_(True)
+    with mode():
+        u = fg.foeed_inpaint_diff(x, m, 0.05, 1.0, 10, 4)
+    assert torch.equal(u.detach(), ref) and calls == (["solve"] if mode is torch.enable_grad else [])
+
+
 def test_kept_states_argument_errors():
     f, m = _image(20, 30, seed=1)
     L, p = fg.lib(), fg._params(0.05, 1.0, 0.0, 4, 3)
