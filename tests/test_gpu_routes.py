@@ -486,6 +486,67 @@ def test_ordered_solve_at_tile_edges(method, shape, sigma):
     assert _kind(method, shape, sigma, 6, 3) == "ordered"
 
 
+# sizes and cycles that run step by step: the autotuner and the graph cache
+
+@pytest.mark.parametrize("method,kw", [(0, {}), (1, {}), (0, dict(diffusivity=1, mu3_mode=1))])
+# under one 64 x 32 tile per SM; one to four (the later triggers too); wide and flat; more than four
+@pytest.mark.parametrize("shape", [(300, 515), (625, 1031), (97, 2111), (1201, 1999)])
+def test_autotuner_on_stepwise_solves(method, kw, shape):
+    """Cycles of one step are timed: the plan says so, the choice is the fastest and is kept, and every tile shape gives
+    the same bits."""
+    f, m = _image(*shape, seed=6)
+    solve = fg.foeed_inpaint if method == 0 else fg.eed_inpaint
+    two = method == 1 or bool(kw)  # 64 x 32 and 64 x 16 tiles only
+    ua, _ = solve(f, m, 0.05, 1.5, 1, 12, **kw)
+    plan = fg.last_tile_plan()
+    assert fg.last_route()["kind"] == "steps" and plan["tuned"] == 1
+    times = {32: plan["us_h32"], 16: plan["us_h16"]}
+    if not two:
+        times.update({64: plan["us_h64"], 8: plan["us_h8"]})
+    assert all(t > 0 for t in times.values())
+    assert plan["us_chosen"] == min(times.values()) == times[plan["tile_h"]]
+    ub, _ = solve(f, m, 0.05, 1.5, 1, 12, **kw)
+    again = fg.last_tile_plan()
+    assert again["tuned"] == 0 and again["tile_h"] == plan["tile_h"] and torch.equal(ua, ub)
+    try:
+        for pol, th in (("h32", 32), ("h16", 16), ("h64", 32 if two else 64), ("h8", 16 if two else 8)):
+            fg.set_tile_policy(pol)
+            u, _ = solve(f, m, 0.05, 1.5, 1, 12, **kw)
+            assert fg.last_tile_plan()["tile_h"] == th and torch.equal(u, ua), pol
+    finally:
+        fg.set_tile_policy("auto")
+
+
+def test_graph_caches_of_two_threads_evict():
+    """Six graph keys per thread, cycles of 130 steps: more than the four entries of a thread's cache."""
+    f, m = _image(64, 96, seed=3)
+    lams = [0.02 * (i + 1) for i in range(6)]
+    ref = {lam: fg.foeed_inpaint(f, m, lam, 1.0, 130, 2)[0].clone() for lam in lams}
+    got, kinds, errors = {}, [], []
+
+    def worker(tid):
+        try:
+            s = torch.cuda.Stream(device=DEV)
+            for rep in range(2):
+                for lam in (lams if tid == 0 else lams[::-1]):
+                    got[tid, rep, lam] = fg.foeed_inpaint(f, m, lam, 1.0, 130, 2, stream=s)[0]
+                    kinds.append(fg.last_route()["kind"])
+            s.synchronize()
+        except Exception as e:  # reported below
+            errors.append(e)
+
+    torch.cuda.synchronize(DEV)
+    ts = [threading.Thread(target=worker, args=(t,)) for t in range(2)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not errors, errors
+    assert len(got) == 24 and set(kinds) == {"steps"}
+    for (tid, rep, lam), u in got.items():
+        assert torch.equal(u, ref[lam]), (tid, rep, lam)
+
+
 def test_differentiable_solve_that_gives_up():
     f, m = _image(300, 400, seed=9)
     grads = []
