@@ -105,10 +105,9 @@ struct CycleArgs64 {
 struct FlowArgs {
     StepArgs<float> s;     // mask, sizes, model, control block, partials
     float *C, *A, *B;      // u^{m,0} and the last iterate; scratch images
-    unsigned int *ticket;  // next (step, tile) of this launch
+    unsigned int *ticket;  // next (step, tile) of this launch; cycles of the solve before it (not written by it)
     int *done;             // per tile: steps of the solve completed
     int n, cycles;         // steps per cycle, cycles of this launch
-    int cycle0;            // cycles of the solve before this launch
     int poll0;             // start of the counters of polls
     float alpha[kCycleMax], alpha_lo[kCycleMax];
 };
