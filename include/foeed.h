@@ -83,7 +83,8 @@ typedef struct {
     int diffusivity;  /* foeed_diffusivity */
     int mu3_mode;     /* foeed_mu3_mode (FOEED only) */
     int init_mode;    /* 0: unknown pixels start at the mean of f over K; 1: at u_inout */
-    int check_every;  /* tol > 0: cycles between host polls of the device stop flag (<= 0: 8) */
+    int check_every;  /* tol > 0: least number of cycles between host polls of the device stop flag (<= 0: 8); the
+                         solve stops by itself, and cycles that share a cooperative launch are polled once */
 } foeed_params;
 
 typedef struct {
@@ -106,7 +107,8 @@ size_t foeed_workspace_bytes(int w, int h, foeed_dtype dtype);
  *              bytes, 256-byte aligned; contents on entry are ignored.
  *   report   may be NULL.
  * Stream-ordered on `stream`; returns after the result is written (the call
- * synchronises `stream` once at the end, and every check_every cycles when tol > 0).
+ * synchronises `stream` once at the end, and every check_every cycles, or after the
+ * launch that holds them, when tol > 0).
  * On return the known pixels of u_inout equal f bitwise.
  * u_inout may alias f.
  */
@@ -316,6 +318,9 @@ foeed_status foeed_inpaint_static(const void *f, const uint8_t *mask, void *u_in
  *     tiles of 64 x 32: four, eight), and of at most 128. Shorter ones run step by step, as do
  *     launches of under four steps on images of 305 to 608 tiles of 64 x 16. foeed_last_route
  *     tells which.
+ *     A cooperative launch keeps the slots of its tiles for up to 4096 steps (2048 in order): at
+ *     sizes that fill the GPU, kernels of other streams wait that long (some 48 ms at 2048 x
+ *     2048). Under a fixed policy they come in between steps.
  * The policy applies to the calling host thread's later calls: foeed_inpaint,
  * eed_inpaint and the batched solvers tune as above; foeed_step, eed_step,
  * foeed_inpaint_static and the forward steps of foeed_inpaint_vjp, which do

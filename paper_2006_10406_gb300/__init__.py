@@ -494,7 +494,15 @@ _FoeedInpaint = None
 
 def foeed_inpaint_diff(f, mask, lam, sigma, cycle_len, max_cycles, tau=0.0, checkpoint_every=16):
     """Differentiable FOEED inpainting (torch.autograd): the gradient of any loss of
-    the result flows back to f through foeed_inpaint_vjp."""
+    the result flows back to f through the hand-written adjoint.
+
+    Where grad mode is on and f requires grad, the call keeps the iterate at the start of
+    every cycle (max_cycles images) from forward to backward, if these and a recomputed
+    cycle (max_cycles + cycle_len) are at most twice the images that checkpoints of
+    checkpoint_every would take in the backward (cycle_len * max_cycles + 1 of them if that
+    is 1, else two for every checkpoint_every steps and checkpoint_every more). Otherwise
+    only f and mask live until the backward, which solves again with those checkpoints, as
+    foeed_inpaint_vjp does."""
     global _FoeedInpaint
     if _FoeedInpaint is None:
         _FoeedInpaint = _autograd_function()

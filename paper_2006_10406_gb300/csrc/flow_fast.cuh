@@ -11,20 +11,20 @@
 // What other CTAs wrote is read through the L2 (cp.async.cg, ld.cg). Waits are bounded, as
 // in cycle_fast.cuh.
 //
-// Saves the launch, fill and drain of every step (5.7 us of a 2048 x 2048 step's 26.5);
-// costs two barriers, the flags and 16% more instructions per tile (what a CTA works out
-// once is worked out per tile, and the tensor stage spills a little at 64 registers).
-// us a step, FOEED (EED), sigma 1.5, one launch per step -> this: 1000 x 1400 12.8 -> 11.9
-// (14.4 -> 13.2), 1536 x 1536 17.4 -> 14.6 (19.1 -> 16.6), 1080 x 1920 15.7 -> 13.4
-// (17.3 -> 15.2), 2048 x 2048 26.5 -> 24.3 (29.4 -> 27.3), 2560 x 2560 38.4 -> 37.4
-// (42.8 -> 41.6); 2160 x 3840 even, 4096 x 4096 91.6 -> 96.2.
+// Saves the launch, fill and drain of every step (5.7 us of a 2048 x 2048 step's 25.8);
+// costs two barriers, the flags and 11% more warp instructions (what a CTA works out once is
+// worked out per tile, and the tensor stage spills a little at 64 registers).
+// us a step, FOEED (EED), sigma 1.5, 20 cycles of 40 steps, one launch per step -> this: 1536 x
+// 1536 16.7 -> 14.1 (17.3 -> 14.7), 1080 x 1920 15.2 -> 12.9 (15.6 -> 13.4), 2048 x 2048 25.8 ->
+// 23.6 (27.1 -> 24.7), 2560 x 2560 37.6 -> 36.5 (39.8 -> 38.2); 2160 x 3840 even, 4096 x 4096
+// 91.6 -> 96.2. Short cycles and launches: use_flow in api.cu.
 // 64 x 16 tiles cost more instructions a pixel but let 0.8 to 1.4 megapixels overlap steps; one
 // launch per step (from 1100 x 1100: this on 64 x 32 tiles) -> 64 x 16 tiles, FOEED sigma 1, sigma 2
 // and EED sigma 2: 704 x 1100 8.12 -> 8.39, 8.63 -> 8.92, 8.65 -> 8.98 (left to the step kernels);
 // 720 x 1280 8.88 -> 8.15, 9.63 -> 8.88, 9.94 -> 9.03; 1000 x 1024 9.61 -> 8.26, 10.53 -> 9.16,
 // 10.78 -> 9.33; 1100 x 1100 10.81 -> 9.44, 11.47 -> 10.51, 11.64 -> 10.67; 1000 x 1400 10.94 ->
 // 10.32, 11.74 -> 11.46, 12.02 -> 11.69; 1200 x 1400 11.42 -> 12.17 (left to 64 x 32 tiles). With
-// the two-float update, sigma 2: 640 x 1024 9.33 -> 9.01, 630 x 1030 9.67 -> 9.32, 704 x 1100
+// the two-float update, sigma 2: 640 x 1024 9.33 -> 9.01, 630 x 1030 9.36 -> 9.35, 704 x 1100
 // 9.34 -> 9.23, 1000 x 1024 11.32 -> 9.65. A step cannot take less than its tile's chain of flags,
 // window, stages and store, some 8 us with four tiles per SM. Up to 608 tiles of 64 x 24 the
 // resident-tile kernel goes first where it is faster (kCycleKinds in api.cu).
